@@ -1531,22 +1531,23 @@ __global__ void __launch_bounds__(1024) jac_offsets_kernel(const int32_t* __rest
 // VJP with one warp per centre atom (the atoms of a molecule run in parallel):
 // each warp writes its centre's contributions to every atom of the molecule
 // into contrib[pair_ptr[m] + (I*M + k)*3 + x]; vjp_reduce_kernel then sums
-// them over the centres I in order.
+// them over the centres I in order. Centres of molecules of more than `most`
+// atoms (most <= mx sizes the buffers) are left to fchl19_vjp_large_kernel.
 constexpr int kWideAtoms = 64;   // molecules whose centres' pairs are summed in kWideWarps shares
-__host__ __device__ __forceinline__ size_t vjp_centre_bytes(int mx, int mxp, int rp) {
-  return (size_t)mxp * 16 + vjp_warp_bytes(mxp, rp) + (mx >= kWideAtoms ? (size_t)mxp * 12 : 0);
+__host__ __device__ __forceinline__ size_t vjp_centre_bytes(int mxp, int rp) {
+  return (size_t)mxp * 16 + vjp_warp_bytes(mxp, rp);
 }
 
 __global__ void __launch_bounds__(32 * kWarpsFwd)
 fchl19_vjp_centre_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem,
-                         const int32_t* __restrict__ mol_ptr, int n_mol, int n_atoms, int mx, int mxp, int rp,
+                         const int32_t* __restrict__ mol_ptr, int n_mol, int n_atoms, int mx, int most, int mxp, int rp,
                          Fchl19Consts c, const float* __restrict__ grad_rep, int rep_ld,
                          const int64_t* __restrict__ pair_ptr, float* __restrict__ contrib, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int atom = blockIdx.x * kWarpsFwd + warp;
   if (atom >= n_atoms) return;
-  char* base = smem_raw + warp * vjp_centre_bytes(mx, mxp, rp);
+  char* base = smem_raw + warp * vjp_centre_bytes(mxp, rp);
   float4* pos = reinterpret_cast<float4*>(base);
   VjpWarp s = carve_vjp(base + (size_t)mxp * 16, mxp, rp);
   const int m = find_molecule(mol_ptr, n_mol, atom);
@@ -1557,53 +1558,26 @@ fchl19_vjp_centre_kernel(const float* __restrict__ coords, const int32_t* __rest
     if (lane == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
     return;
   }
+  if (M > most) return;
   stage_molecule(coords, elem, a0, M, c.n_el, pos, lane, 32, err);
+  for (int k = lane; k < 3 * M; k += 32) s.facc[k] = 0.0f;
+  __syncwarp();
+  vjp_centre(pos, M, il, c, grad_rep + (size_t)atom * rep_ld, s, lane);
+  __syncwarp();
   float* out = contrib + pair_ptr[m] + (long)il * M * 3;
-  if (M < kWideAtoms) {
-    for (int k = lane; k < 3 * M; k += 32) s.facc[k] = 0.0f;
-    __syncwarp();
-    vjp_centre(pos, M, il, c, grad_rep + (size_t)atom * rep_ld, s, lane);
-    __syncwarp();
-    for (int k = lane; k < 3 * M; k += 32) out[k] = s.facc[k];
-    return;
-  }
-  // a molecule of the CTA-per-centre kernel's sizes: the same shares, one after
-  // the other, and the same sum over them, so that its forces do not depend on
-  // the kernel its batch selects
-  float* total = reinterpret_cast<float*>(base + (size_t)mxp * 16 + vjp_warp_bytes(mxp, rp));
-  load_grad_row(s.g, grad_rep + (size_t)atom * rep_ld, c, lane);
-  const int n = neighbour_list(pos, M, il, c, s.nb_u, s.nb_2b, s.nb_el, s.nb_idx, lane);
-  for (int w = 0; w < kWideWarps; ++w) {
-    for (int k = lane; k < 3 * M; k += 32) s.facc[k] = 0.0f;
-    __syncwarp();
-    vjp_from_neighbours<true>(n, il, c, s, lane, w, kWideWarps);
-    __syncwarp();
-    for (int k = lane; k < 3 * M; k += 32) total[k] = w == 0 ? s.facc[k] : total[k] + s.facc[k];
-    __syncwarp();
-  }
-  for (int k = lane; k < 3 * M; k += 32) out[k] = total[k];
+  for (int k = lane; k < 3 * M; k += 32) out[k] = s.facc[k];
 }
 
-// The same with a CTA per centre (small batches of molecules with many
-// neighbours, where one warp per centre leaves most of the chip waiting for the
-// largest molecules): the warps share the neighbour list and the gradient row,
-// take the pairs' chunks in turn into accumulators of their own, and the CTA
-// adds those in warp order.
-__global__ void __launch_bounds__(32 * kWideWarps)
-fchl19_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem,
-                       const int32_t* __restrict__ mol_ptr, int n_mol, int mx, int mxp, int rp, Fchl19Consts c,
-                       const float* __restrict__ grad_rep, int rep_ld, const int64_t* __restrict__ pair_ptr,
-                       float* __restrict__ contrib, int* err) {
+// One centre by a CTA (one warp would leave most of the chip waiting for the
+// centres with the most neighbours): the warps share the neighbour list and the
+// gradient row, take the pairs' chunks in turn into accumulators of their own, and
+// the CTA adds those in warp order.
+__device__ __forceinline__ void vjp_wide_centre(const float* __restrict__ coords, const int32_t* __restrict__ elem,
+                                                int a0, int M, int il, int mxp, int rp, const Fchl19Consts& c,
+                                                const float* __restrict__ grad_rep, int rep_ld,
+                                                float* __restrict__ out, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, atom = blockIdx.x;
-  const int m = find_molecule(mol_ptr, n_mol, atom);
-  const int a0 = __ldg(mol_ptr + m);
-  const int M = __ldg(mol_ptr + m + 1) - a0;
-  const int il = atom - a0;
-  if (M > mx) {
-    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
-    return;
-  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float4* pos = reinterpret_cast<float4*>(smem_raw);
   VjpWarp s;
   s.stage = nullptr;
@@ -1615,7 +1589,7 @@ fchl19_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restri
   float* facc = reinterpret_cast<float*>(s.nb_idx + mxp);   // [kWideWarps][3 mxp]
   s.facc = facc + (size_t)warp * 3 * mxp;
   stage_molecule(coords, elem, a0, M, c.n_el, pos, threadIdx.x, blockDim.x, err);
-  const float* grow = grad_rep + (size_t)atom * rep_ld;
+  const float* grow = grad_rep + (size_t)(a0 + il) * rep_ld;
   const int sh = c.base3 & 1;   // the layout of load_grad_row
   for (int k = threadIdx.x; k < c.rep_dim; k += blockDim.x) s.g[k + (k >= c.base3 ? sh : 0)] = __ldg(grow + k);
   for (int k = lane; k < 3 * M; k += 32) s.facc[k] = 0.0f;
@@ -1625,11 +1599,92 @@ fchl19_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restri
   const int parts = M < kWideAtoms ? 1 : kWideWarps;   // small molecules: one warp, the order of the other kernel
   if (warp < parts) vjp_from_neighbours<true>(n, il, c, s, lane, warp, parts);
   __syncthreads();
-  float* out = contrib + pair_ptr[m] + (long)il * M * 3;
   for (int k = threadIdx.x; k < 3 * M; k += blockDim.x) {
     float sum = facc[k];
     for (int w = 1; w < parts; ++w) sum += facc[(size_t)w * 3 * mxp + k];
     out[k] = sum;
+  }
+}
+
+// Every centre by a CTA: batches of few atoms, or of molecules that are large in the mean.
+__global__ void __launch_bounds__(32 * kWideWarps)
+fchl19_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem,
+                       const int32_t* __restrict__ mol_ptr, int n_mol, int mx, int mxp, int rp, Fchl19Consts c,
+                       const float* __restrict__ grad_rep, int rep_ld, const int64_t* __restrict__ pair_ptr,
+                       float* __restrict__ contrib, int* err) {
+  const int atom = blockIdx.x;
+  const int m = find_molecule(mol_ptr, n_mol, atom);
+  const int a0 = __ldg(mol_ptr + m);
+  const int M = __ldg(mol_ptr + m + 1) - a0;
+  if (M > mx) {
+    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
+    return;
+  }
+  vjp_wide_centre(coords, elem, a0, M, atom - a0, mxp, rp, c, grad_rep, rep_ld,
+                  contrib + pair_ptr[m] + (long)(atom - a0) * M * 3, err);
+}
+
+// The centres of the molecules of kWideAtoms atoms or more alone, beside a
+// warp-per-centre launch for the others: a fixed number of CTAs look through the
+// molecules' sizes (2048 at a time, past a group without a large one in one
+// barrier) and take the large centres in turn. With the large molecules in the
+// warp-per-centre kernel, a warp walked the ~10 000 pairs of a centre of a 200-atom
+// molecule in eight shares, and every warp held their accumulators: ten molecules of
+// 150-200 atoms among 300 small ones 1167 us for the call, now 491; 300 molecules of
+// 30-63 atoms with room for 200 719 us, now 435 (two CTAs per SM, now seven).
+constexpr int kLargeCtasPerSm = 4;   // 59 registers: 4 CTAs of 256 threads per SM
+constexpr int kLargeGroup = 8;       // rounds of 256 molecules per look
+
+__global__ void __launch_bounds__(32 * kWideWarps, kLargeCtasPerSm)
+fchl19_vjp_large_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem,
+                        const int32_t* __restrict__ mol_ptr, int n_mol, int mx, int mxp, int rp, Fchl19Consts c,
+                        const float* __restrict__ grad_rep, int rep_ld, const int64_t* __restrict__ pair_ptr,
+                        float* __restrict__ contrib, int* err) {
+  constexpr int T = 32 * kWideWarps;
+  __shared__ int upto[T], wsum[kWideWarps];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto large = [&](int m) {   // centres of molecule m for this kernel (sizes above mx are recorded by the other)
+    const int M = m < n_mol ? __ldg(mol_ptr + m + 1) - __ldg(mol_ptr + m) : 0;
+    return M >= kWideAtoms && M <= mx ? M : 0;
+  };
+  long next = blockIdx.x, before = 0;   // this CTA's next large centre; large centres of earlier rounds
+  for (int base = 0; base < n_mol; base += kLargeGroup * T) {
+    int any = 0;
+#pragma unroll
+    for (int u = 0; u < kLargeGroup; ++u) any |= large(base + u * T + tid);
+    if (!__syncthreads_or(any)) continue;
+#pragma unroll 1
+    for (int u = 0; u < kLargeGroup; ++u) {
+      const int m0 = base + u * T;
+      int incl = large(m0 + tid);
+      if (!__syncthreads_or(incl)) continue;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) wsum[warp] = incl;
+      __syncthreads();
+      for (int w = 0; w < warp; ++w) incl += wsum[w];
+      upto[tid] = incl;
+      __syncthreads();
+      const int total = upto[T - 1];
+      for (; next < before + total; next += gridDim.x) {
+        const int at = (int)(next - before);
+        int lo = 0, hi = T - 1;   // first molecule of the round with upto > at
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (upto[mid] > at) hi = mid;
+          else lo = mid + 1;
+        }
+        const int m = m0 + lo, il = at - (lo > 0 ? upto[lo - 1] : 0);
+        const int a0 = __ldg(mol_ptr + m), M = __ldg(mol_ptr + m + 1) - a0;
+        vjp_wide_centre(coords, elem, a0, M, il, mxp, rp, c, grad_rep, rep_ld,
+                        contrib + pair_ptr[m] + (long)il * M * 3, err);
+        __syncthreads();   // the centre's buffers are read
+      }
+      before += total;
+    }
   }
 }
 
@@ -2151,18 +2206,26 @@ extern "C" int qmlr_fchl19_vjp_atoms(const float* coords, const int32_t* elem, c
   const int rp = rep_pad_of(rd);
   const int mx = max_mol_atoms;
   const int mxp = (mx + 3) & ~3;
-  const size_t smem = kWarpsFwd * vjp_centre_bytes(mx, mxp, rp);
-  QMLR_REQUIRE(smem <= 227 * 1024, "shared memory request too large");
-  QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_vjp_centre_kernel, 227 * 1024));
+  QMLR_REQUIRE(kWarpsFwd * vjp_centre_bytes(mxp, rp) <= 227 * 1024, "shared memory request too large");
   cudaStream_t st = as_stream(stream);
-  if (wide_atoms(mx, n_mol, n_atoms) && vjp_wide_smem_bytes(mxp, rp) <= 227 * 1024) {
+  const size_t wide = vjp_wide_smem_bytes(mxp, rp);   // below the size required above
+  if (wide_atoms(mx, n_mol, n_atoms)) {
     QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_vjp_wide_kernel, 227 * 1024));
-    fchl19_vjp_wide_kernel<<<n_atoms, 32 * kWideWarps, vjp_wide_smem_bytes(mxp, rp), st>>>(
+    fchl19_vjp_wide_kernel<<<n_atoms, 32 * kWideWarps, wide, st>>>(
         coords, elem, mol_ptr, n_mol, mx, mxp, rp, c, grad_rep, rep_ld, pair_ptr, contrib, device_error_ptr());
   } else {
-    fchl19_vjp_centre_kernel<<<(n_atoms + kWarpsFwd - 1) / kWarpsFwd, 32 * kWarpsFwd, smem, st>>>(
-        coords, elem, mol_ptr, n_mol, n_atoms, mx, mxp, rp, c, grad_rep, rep_ld, pair_ptr, contrib,
+    const int most = std::min(mx, kWideAtoms - 1), mp = (most + 3) & ~3;
+    QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_vjp_centre_kernel, 227 * 1024));
+    fchl19_vjp_centre_kernel<<<(n_atoms + kWarpsFwd - 1) / kWarpsFwd, 32 * kWarpsFwd,
+                               kWarpsFwd * vjp_centre_bytes(mp, rp), st>>>(
+        coords, elem, mol_ptr, n_mol, n_atoms, mx, most, mp, rp, c, grad_rep, rep_ld, pair_ptr, contrib,
         device_error_ptr());
+    if (mx >= kWideAtoms) {
+      QMLR_LAUNCH_CHECK();
+      QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_vjp_large_kernel, 224 * 1024));
+      fchl19_vjp_large_kernel<<<std::min(n_atoms, kLargeCtasPerSm * sm_count()), 32 * kWideWarps, wide, st>>>(
+          coords, elem, mol_ptr, n_mol, mx, mxp, rp, c, grad_rep, rep_ld, pair_ptr, contrib, device_error_ptr());
+    }
   }
   QMLR_LAUNCH_CHECK();
   if (mx >= kWideAtoms)
