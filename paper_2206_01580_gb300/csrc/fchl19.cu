@@ -1632,7 +1632,7 @@ fchl19_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restri
 // molecule in eight shares, and every warp held their accumulators: ten molecules of
 // 150-200 atoms among 300 small ones 1167 us for the call, now 491; 300 molecules of
 // 30-63 atoms with room for 200 719 us, now 435 (two CTAs per SM, now seven).
-constexpr int kLargeCtasPerSm = 4;   // 59 registers: 4 CTAs of 256 threads per SM
+constexpr int kLargeCtasPerSm = 4;   // 64 registers: 4 CTAs of 256 threads per SM
 constexpr int kLargeGroup = 8;       // rounds of 256 molecules per look
 
 __global__ void __launch_bounds__(32 * kWideWarps, kLargeCtasPerSm)
@@ -1693,44 +1693,80 @@ __host__ __device__ __forceinline__ size_t vjp_wide_smem_bytes(int mxp, int rp) 
 }
 
 // grad[k][x] = scale * sum_{I = 0..M-1} contrib[pair_ptr[m] + (I*M + k_local)*3 + x] (+ grad if accumulate).
-// LANES = 8: the centres of a molecule of kWideAtoms atoms or more are shared by
-// eight lanes (lane l adds l, l + 8, ..., then a fixed tree); smaller molecules
-// are added in order by one. One thread per (atom, axis) walked the centres of
-// 200-atom molecules in 25 us (8 us now); eight lanes on 18-atom molecules take
-// 72 us instead of 22 (212 k atoms), so launches that can hold no large
-// molecule run LANES = 1. The order depends on M alone. Sixteen loads stand in
-// flight (a 21-atom molecule 7.6 us with four, now 4.2).
+// The centres of a molecule of kWideAtoms atoms or more are shared by eight lanes
+// (lane l adds l, l + 8, ..., then a fixed tree); smaller molecules are added in
+// order by one. The order depends on M alone. Sixteen loads stand in flight (a
+// 21-atom molecule 7.6 us with four, now 4.2).
+// LANES = 8 gives every output its eight lanes: one thread per (atom, axis) walked
+// the centres of 200-atom molecules in 25 us (8 us now). LANES = 1 gives it one, and
+// the lanes of a warp that meets outputs of large molecules share those, four at a
+// time; that is the better form where small molecules fill the chip by themselves
+// (216 k atoms in 18-atom molecules 128 us with eight lanes, 17 with one; 12 600 atoms
+// 9.7 and 4.3; 18 000 atoms in 180-atom molecules 10.3 and 19.9).
 constexpr int kReduceLoads = 16;
+
+__device__ __forceinline__ float reduce_run(const float* __restrict__ cp, int M, int first, int step) {
+  float sum = 0.f;
+  for (int i0 = first; i0 < M; i0 += kReduceLoads * step) {   // loads in flight, then the sum in order
+    float v[kReduceLoads];
+#pragma unroll
+    for (int q = 0; q < kReduceLoads; ++q) {
+      const int I = i0 + q * step;
+      v[q] = I < M ? __ldg(cp + (long)I * M * 3) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kReduceLoads; ++q)
+      if (i0 + q * step < M) sum += v[q];
+  }
+  return sum;
+}
 
 template <int LANES>
 __global__ void __launch_bounds__(256)
 vjp_reduce_kernel(const int32_t* __restrict__ mol_ptr, int n_mol, int n_atoms, const int64_t* __restrict__ pair_ptr,
                   const float* __restrict__ contrib, float scale, int accumulate, float* __restrict__ grad) {
-  const int t = (blockIdx.x * 256 + threadIdx.x) / LANES, l = threadIdx.x % LANES;
-  float sum = 0.f;
+  const int t = (blockIdx.x * 256 + threadIdx.x) / LANES, l = threadIdx.x & 7;
+  const float* cp = contrib;   // this thread's output: its first term and the molecule's size
+  int M = 0;
   if (t < 3 * n_atoms) {
-    const int atom = t / 3, x = t % 3;
+    const int atom = t / 3;
     const int m = find_molecule(mol_ptr, n_mol, atom);
-    const int a0 = __ldg(mol_ptr + m), M = __ldg(mol_ptr + m + 1) - a0, kl = atom - a0;
-    const float* cp = contrib + pair_ptr[m] + (long)kl * 3 + x;
-    const int step = LANES > 1 && M >= kWideAtoms ? LANES : 1;
-    if (l < step) {
-      for (int i0 = l; i0 < M; i0 += kReduceLoads * step) {   // loads in flight, then the sum in order
-        float v[kReduceLoads];
+    const int a0 = __ldg(mol_ptr + m);
+    M = __ldg(mol_ptr + m + 1) - a0;
+    cp += pair_ptr[m] + (long)(atom - a0) * 3 + t % 3;
+  }
+  float sum = 0.f;
+  if constexpr (LANES == 8) {
+    if (M >= kWideAtoms) sum = reduce_run(cp, M, l, 8);
+    else if (l == 0) sum = reduce_run(cp, M, 0, 1);
 #pragma unroll
-        for (int q = 0; q < kReduceLoads; ++q) {
-          const int I = i0 + q * step;
-          v[q] = I < M ? __ldg(cp + (long)I * M * 3) : 0.f;
-        }
+    for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (l > 0) return;
+  } else {
+    if (M < kWideAtoms) sum = reduce_run(cp, M, 0, 1);
+    const int lane = threadIdx.x & 31;
+    for (unsigned large = __ballot_sync(0xffffffffu, M >= kWideAtoms); large;) {
+      int src = -1;   // the output that this lane's group of eight takes
 #pragma unroll
-        for (int q = 0; q < kReduceLoads; ++q)
-          if (i0 + q * step < M) sum += v[q];
+      for (int g = 0; g < 4; ++g) {
+        if (g == lane >> 3 && large) src = __ffs(large) - 1;
+        large &= large - 1u;
+      }
+      const int from = max(src, 0);
+      const float* p = reinterpret_cast<const float*>(
+          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cp), from));
+      const int size = __shfl_sync(0xffffffffu, M, from);
+      float part = src >= 0 ? reduce_run(p, size, l, 8) : 0.f;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const float v = __shfl_sync(0xffffffffu, part, 8 * g);
+        if (__shfl_sync(0xffffffffu, src, 8 * g) == lane) sum = v;
       }
     }
   }
-#pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (t < 3 * n_atoms && l == 0) grad[t] = accumulate ? grad[t] + scale * sum : scale * sum;
+  if (t < 3 * n_atoms) grad[t] = accumulate ? grad[t] + scale * sum : scale * sum;
 }
 
 // ---------------------------------------------------------------------------
@@ -2209,7 +2245,8 @@ extern "C" int qmlr_fchl19_vjp_atoms(const float* coords, const int32_t* elem, c
   QMLR_REQUIRE(kWarpsFwd * vjp_centre_bytes(mxp, rp) <= 227 * 1024, "shared memory request too large");
   cudaStream_t st = as_stream(stream);
   const size_t wide = vjp_wide_smem_bytes(mxp, rp);   // below the size required above
-  if (wide_atoms(mx, n_mol, n_atoms)) {
+  const bool all_wide = wide_atoms(mx, n_mol, n_atoms);
+  if (all_wide) {
     QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_vjp_wide_kernel, 227 * 1024));
     fchl19_vjp_wide_kernel<<<n_atoms, 32 * kWideWarps, wide, st>>>(
         coords, elem, mol_ptr, n_mol, mx, mxp, rp, c, grad_rep, rep_ld, pair_ptr, contrib, device_error_ptr());
@@ -2228,7 +2265,7 @@ extern "C" int qmlr_fchl19_vjp_atoms(const float* coords, const int32_t* elem, c
     }
   }
   QMLR_LAUNCH_CHECK();
-  if (mx >= kWideAtoms)
+  if (mx >= kWideAtoms && (all_wide || 24L * n_atoms <= 1024L * sm_count()))   // large in the mean, or all at once
     vjp_reduce_kernel<8><<<(3 * n_atoms + 31) / 32, 256, 0, st>>>(mol_ptr, n_mol, n_atoms, pair_ptr, contrib, scale,
                                                                  accumulate, grad_coords);
   else

@@ -79,3 +79,38 @@ def test_buffers_for_large_molecules_cost_the_others_little(q):
     g = torch.ones((len(elem), q.rep_ld_of(p.rep_dim)), device="cuda")
     t = [_microseconds(lambda: q.fchl19_vjp_atoms(coords, elem, ptr, mx, p, g)) for mx in (63, 200)]
     assert t[1] <= 1.25 * t[0], t
+
+
+@pytest.mark.parametrize("n_small", [1000, 20000])
+def test_large_molecules_among_pairs(q, n_small):
+    """The reduction with eight lanes per output and with one: warps with outputs of small, of large
+    and of both kinds of molecules; each large molecule keeps the bits that it has alone."""
+    rng = np.random.default_rng(n_small)
+    p = from_table("EF", n2=24, n3=22)
+    sizes = np.full(n_small, 2)
+    sizes[[0, 7, 8, 500, n_small - 2]] = 66, 64, 200, 63, 91
+    mols = [_grid_molecule(rng, n) for n in sizes]
+    ptr = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    coords = np.concatenate([x for x, _ in mols]).astype(np.float32)
+    elem = np.concatenate([e for _, e in mols])
+    g = torch.as_tensor(rng.normal(size=(len(elem), q.rep_ld_of(p.rep_dim))).astype(np.float32)).cuda()
+    got = q.fchl19_vjp_atoms(coords, elem, ptr, 200, p, g)
+    for k in [0, 1, 6, 7, 8, 9, 500, n_small - 2, n_small - 1]:
+        at = slice(int(ptr[k]), int(ptr[k + 1]))
+        want = q.fchl19_vjp_atoms(coords[at], elem[at], np.array([0, sizes[k]], np.int32), 200, p, g[at].contiguous())
+        assert torch.equal(got[at], want)
+    assert q.device_status() == 0
+
+
+def test_reduction_of_small_molecules_with_room_for_large_ones(q):
+    """12 000 molecules of 18 atoms with room for 200 against room for 29: the same centres and sums, beside a look
+    at 12 000 sizes and a launch, ~10 us of ~1 ms. A quarter is allowed."""
+    rng = np.random.default_rng(2)
+    p = from_table("EF", n2=24, n3=22)
+    mols = [_grid_molecule(rng, 18) for _ in range(12000)]
+    ptr = torch.as_tensor((18 * np.arange(12001)).astype(np.int32)).cuda()
+    coords = torch.as_tensor(np.concatenate([x for x, _ in mols]).astype(np.float32)).cuda()
+    elem = torch.as_tensor(np.concatenate([e for _, e in mols])).cuda()
+    g = torch.ones((len(elem), q.rep_ld_of(p.rep_dim)), device="cuda")
+    t = [_microseconds(lambda: q.fchl19_vjp_atoms(coords, elem, ptr, mx, p, g)) for mx in (29, 200)]
+    assert t[1] <= 1.25 * t[0], t
