@@ -339,10 +339,10 @@ __device__ __forceinline__ void reduce_scatter_step(float (&v)[D], int lane) {
 
 // The chains, phases and products run on packed pairs (half the instructions of
 // the scalar form, which missed the instruction cache: 1.2 of 3.0 stall cycles
-// per issue at D = 128), and the phases and weights are read stack-minor at a
-// uniform row address plus the stack. 53 k atoms at N_F = 16384, energies only:
-// 1.39 -> 1.13 ms.
-template <int D, bool GRAD>
+// per issue at D = 128), and the phases and weights are read at a uniform row
+// address plus the stack's offset (MINOR: stack-minor order, coalesced; else the
+// natural order). 53 k atoms at N_F = 16384, energies only: 1.39 -> 1.13 ms.
+template <int D, bool GRAD, bool MINOR>
 __global__ void __launch_bounds__(kStacksPerCta, GRAD ? 2 : 3)
 sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
   constexpr int W = (D + 31) / 32;
@@ -374,13 +374,15 @@ sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
   if (active) {
     const f32x2 scale = pack2(a.scale, a.scale);
     const float gs = -a.pref * a.scale;
+    const int at = MINOR ? s : s * D;
+    const long step = MINOR ? a.n_stack : 1;
 #pragma unroll
     for (int i = 0; i < D; i += 2) {
-      const float* bi = a.b + (long)i * a.n_stack;      // uniform
-      const float* ai = a.alpha + (long)i * a.n_stack;
-      const float al0 = __ldg(ai + s), al1 = __ldg(ai + a.n_stack + s);
+      const float* bi = a.b + i * step;      // uniform
+      const float* ai = a.alpha + i * step;
+      const float al0 = __ldg(ai + at), al1 = __ldg(ai + step + at);
       float r0, r1;
-      unpack2(reduce_phase2(fma2(v[i / 2], scale, pack2(__ldg(bi + s), __ldg(bi + a.n_stack + s)))), r0, r1);
+      unpack2(reduce_phase2(fma2(v[i / 2], scale, pack2(__ldg(bi + at), __ldg(bi + step + at)))), r0, r1);
       e = fmaf(al0, __cosf(r0), e);
       e = fmaf(al1, __cosf(r1), e);
       if (GRAD) v[i / 2] = mul2(mul2(pack2(gs, gs), pack2(al0, al1)), pack2(__sinf(r0), __sinf(r1)));
@@ -498,30 +500,35 @@ int sorf_segment_energy(const double* atom_e, int n_part, int n_atoms, const int
   return segment_energy_launch(atom_e, n_part, n_atoms, mol_ptr, n_mol, E, s);
 }
 
-template <int D, bool GRAD>
+template <int D, bool GRAD, bool MINOR>
 static int launch_atoms(const SorfArgs& a, double* atom_e, int n_mol, double* E, cudaStream_t s) {
   const int nt = std::min(kStacksPerCta, ((a.n_stack + 31) / 32) * 32);
   constexpr int W = (D + 31) / 32;
   const size_t smem = (size_t)(D + 4) * 4 + (kStacksPerCta / 32) * 8 + (size_t)4 * W * kStacksPerCta * 4 +
                       (GRAD ? (D >= 32 ? (size_t)(kStacksPerCta / 32) * D * 4 : (size_t)nt * (D + 1) * 4) : 0);
-  QMLR_CUDA_TRY(smem_attr_once((const void*)sorf_atom_kernel<D, GRAD>, 227 * 1024));
+  QMLR_CUDA_TRY(smem_attr_once((const void*)sorf_atom_kernel<D, GRAD, MINOR>, 227 * 1024));
   if (a.n_atoms > 0) {
     dim3 grid(a.n_atoms, a.n_part);
-    sorf_atom_kernel<D, GRAD><<<grid, nt, smem, s>>>(a, atom_e);
+    sorf_atom_kernel<D, GRAD, MINOR><<<grid, nt, smem, s>>>(a, atom_e);
     QMLR_LAUNCH_CHECK();
   }
   return segment_energy_launch(atom_e, a.n_part, a.n_atoms, a.mol_ptr, n_mol, E, s);
 }
 
-// Energies and (optionally) gradients, atoms in parallel. Internal entry used
-// by qmlr_sorf_grad and the model's prediction (b and alpha stack-minor).
-int sorf_energy_atoms(const SorfArgs& a, int d, double* atom_e, int n_mol, double* E, bool grad,
-                      cudaStream_t s) {
+template <int D, bool MINOR>
+static int launch_atoms(const SorfArgs& a, double* atom_e, int n_mol, double* E, bool grad, cudaStream_t s) {
+  return grad ? launch_atoms<D, true, MINOR>(a, atom_e, n_mol, E, s) : launch_atoms<D, false, MINOR>(a, atom_e, n_mol, E, s);
+}
+
+// Energies and (optionally) gradients, atoms in parallel. Internal entry used by
+// qmlr_sorf_grad and the model's prediction (MINOR: b and alpha stack-minor).
+template <bool MINOR>
+static int sorf_energy_atoms(const SorfArgs& a, int d, double* atom_e, int n_mol, double* E, bool grad, cudaStream_t s) {
   switch (d) {
-    case 16: return grad ? launch_atoms<16, true>(a, atom_e, n_mol, E, s) : launch_atoms<16, false>(a, atom_e, n_mol, E, s);
-    case 32: return grad ? launch_atoms<32, true>(a, atom_e, n_mol, E, s) : launch_atoms<32, false>(a, atom_e, n_mol, E, s);
-    case 64: return grad ? launch_atoms<64, true>(a, atom_e, n_mol, E, s) : launch_atoms<64, false>(a, atom_e, n_mol, E, s);
-    default: return grad ? launch_atoms<128, true>(a, atom_e, n_mol, E, s) : launch_atoms<128, false>(a, atom_e, n_mol, E, s);
+    case 16: return launch_atoms<16, MINOR>(a, atom_e, n_mol, E, grad, s);
+    case 32: return launch_atoms<32, MINOR>(a, atom_e, n_mol, E, grad, s);
+    case 64: return launch_atoms<64, MINOR>(a, atom_e, n_mol, E, grad, s);
+    default: return launch_atoms<128, MINOR>(a, atom_e, n_mol, E, grad, s);
   }
 }
 
@@ -553,7 +560,7 @@ int sorf_energy_grad_model(const float* x, int d, const int32_t* mol_ptr, int n_
                            const uint32_t* sign_bits, int T, const float* bT, int n_features, double sigma,
                            const float* alphaT, double* atom_e, double* E, float* gx, cudaStream_t s) {
   SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, bT, n_features, sigma, alphaT, gx);
-  return sorf_energy_atoms(a, d, atom_e, n_mol, E, gx != nullptr, s);
+  return sorf_energy_atoms<true>(a, d, atom_e, n_mol, E, gx != nullptr, s);
 }
 
 template <int D>
@@ -728,6 +735,9 @@ extern "C" int qmlr_force_rows(const float* tangents, int32_t d, const int64_t* 
   }
 }
 
+// Atoms up to which qmlr_sorf_grad reads b and alpha in place.
+static constexpr int kSorfNaturalAtoms = 128;
+
 extern "C" int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr, int32_t n_mol,
                               int32_t n_atoms, const uint32_t* sign_bits, int32_t T, const float* b,
                               int32_t n_features, double sigma, const float* alpha, double* atom_energy,
@@ -740,25 +750,37 @@ extern "C" int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr,
   if (n_mol == 0) return QMLR_OK;
   QMLR_REQUIRE(mol_ptr && energies && atom_energy, "NULL pointer argument");
   QMLR_REQUIRE(n_atoms == 0 || (x && sign_bits && b && alpha), "NULL pointer argument");
-  // phases and weights in stack-minor order for coalesced loads (stream-ordered
-  // scratch): read in natural order each load touched 32 lines, 422 us of E + F
-  // for a 3000-atom periodic cell at N_F = 16384
+  // Phases and weights in stack-minor order (stream-ordered scratch) for coalesced
+  // loads: in natural order each load touches 32 lines, 422 us of E + F for a
+  // 3000-atom periodic cell at N_F = 16384. Natural order where the scratch and its
+  // launch cost more than the loads (a call of up to 128 atoms 27-33 us at 512 to 16384
+  // features, with the scratch 33-36; from 150 atoms on the scratch wins), under
+  // capture (a graph that owns memory has fewer uses), and when there is no memory for
+  // it; the results have the same bits.
   cudaStream_t st = as_stream(stream);
   float* bT = nullptr;
-  QMLR_CUDA_TRY(cudaMallocAsync(&bT, sizeof(float) * 2 * (size_t)n_features, st));
-  int rc = QMLR_OK;
-  if (n_atoms > 0) {
-    transpose_phases_kernel<<<(n_features + 255) / 256, 256, 0, st>>>(b, alpha, d, n_features / d, bT, bT + n_features);
-    count_launch();
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      set_error("kernel launch failed: %s", cudaGetErrorString(e));
-      rc = QMLR_ECUDA;
+  if (n_atoms > kSorfNaturalAtoms) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+        cudaMallocAsync(&bT, sizeof(float) * 2 * (size_t)n_features, st) != cudaSuccess) {
+      bT = nullptr;
+      cudaGetLastError();
     }
   }
-  if (rc == QMLR_OK) {
-    SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, bT, n_features, sigma, bT + n_features, gx);
-    rc = sorf_energy_atoms(a, d, atom_energy, n_mol, energies, gx != nullptr, st);
+  if (bT == nullptr) {
+    const SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, b, n_features, sigma, alpha, gx);
+    return sorf_energy_atoms<false>(a, d, atom_energy, n_mol, energies, gx != nullptr, st);
+  }
+  transpose_phases_kernel<<<(n_features + 255) / 256, 256, 0, st>>>(b, alpha, d, n_features / d, bT, bT + n_features);
+  count_launch();
+  int rc = QMLR_OK;
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("kernel launch failed: %s", cudaGetErrorString(e));
+    rc = QMLR_ECUDA;
+  } else {
+    const SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, bT, n_features, sigma, bT + n_features, gx);
+    rc = sorf_energy_atoms<true>(a, d, atom_energy, n_mol, energies, gx != nullptr, st);
   }
   cudaFreeAsync(bT, st);
   return rc;
