@@ -635,13 +635,16 @@ typedef struct qmlr_solve_opts {
  * (two-sum) folded into FP64 every 128 terms, i.e. about twice FP32's
  * precision (relative error ~1e-12 of the sum of |terms| on feature data);
  * fixed summation order, so repeated calls agree bitwise. work: device scratch
- * of qmlr_normal_apply_workspace_bytes bytes, 256-byte aligned. Asynchronous.
+ * of qmlr_normal_apply_workspace_bytes bytes, 256-byte aligned; 8 N_F bytes per
+ * 2048 rows in place of the 8 N_F per 128 rows in that size are enough (the same
+ * result, fewer CTAs). Asynchronous.
  */
 int64_t qmlr_normal_apply_workspace_bytes(int64_t n_rows, int32_t n_features);
 int qmlr_normal_apply(const float* Z, int64_t n_rows, int32_t n_features, int64_t ldz, double lambda,
                       const double* p, double* q, void* work, int64_t work_bytes, void* stream);
 
-/* Device workspace bytes of qmlr_gram_solve. */
+/* Device workspace bytes of qmlr_gram_solve. 8 N_F bytes per 2048 rows in place of
+ * the 8 N_F per 128 rows in that size are enough, as for qmlr_normal_apply. */
 int64_t qmlr_solve_workspace_bytes(int64_t n_rows, int32_t n_features);
 
 /*

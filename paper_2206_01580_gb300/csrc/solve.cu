@@ -1323,22 +1323,28 @@ zmv4_kernel(const float* __restrict__ Z, long n_rows, int n_features, long ldz, 
 // the weights at N_F = 16384, so it depends on n_rows alone, not on how many
 // folds a CTA takes. Enough CTAs for ~16 of 128 threads per SM, 512 features
 // each (one CTA per 2048 rows and 256 features left 6000 x 2048 with 24 CTAs).
+// A workspace that holds one sum per 2048 rows only is enough too: a CTA then walks
+// those rows and writes their sum, the same additions in fewer CTAs (Z^T t of
+// 6000 x 2048 128 us instead of 14, of 40 000 x 16384 438 instead of 390).
 constexpr int kPartFolds = 16;
 constexpr int kZtThreads = 128, kZtCols = 4 * kZtThreads;
 
 static int64_t zt_folds(int64_t n_rows) { return std::max<int64_t>((n_rows + kFold - 1) / kFold, 1); }
+static int64_t zt_parts(int64_t n_rows) { return (zt_folds(n_rows) + kPartFolds - 1) / kPartFolds; }
 
-// folds[b][f] = sum over fold b's rows r of Z[r][f] t[r]. A thread owns four
+// folds[b][f] = sum over fold b's rows r of Z[r][f] t[r] (PARTS: folds[p][f] = the sum
+// over part p's folds, per_cta = kPartFolds of them). A thread owns four
 // features (VEC: one 16-byte load per row, 8 to 16 rows in flight); t's pairs of a
 // fold are staged in shared memory, one 8-byte broadcast per row and four
 // products (read from global memory per product they cost two of three loads).
-template <bool VEC>
+template <bool VEC, bool PARTS>
 __global__ void __launch_bounds__(kZtThreads)
 ztmv_folds_kernel(const float* __restrict__ Z, long n_rows, int n_features, long ldz, const float* __restrict__ th,
                   const float* __restrict__ tl, int per_cta, double* __restrict__ folds) {
   __shared__ float2 ts[kFold];
   const int f = (blockIdx.x * kZtThreads + threadIdx.x) * 4;
   const long b0 = (long)blockIdx.y * per_cta;
+  [[maybe_unused]] double part[4] = {0.0, 0.0, 0.0, 0.0};
   for (long b = b0; b < b0 + per_cta && b * kFold < n_rows; ++b) {
     const long rb = b * kFold;
     const int cnt = (int)min((long)kFold, n_rows - rb);
@@ -1385,43 +1391,50 @@ ztmv_folds_kernel(const float* __restrict__ Z, long n_rows, int n_features, long
       add(i0 + 8, vb);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (f + k < n_features) folds[b * n_features + f + k] = fold2(s[k], c[k]);
+    for (int k = 0; k < 4; ++k) {
+      if (PARTS) part[k] += fold2(s[k], c[k]);
+      else if (f + k < n_features) folds[b * n_features + f + k] = fold2(s[k], c[k]);
+    }
   }
+  if (PARTS)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (f + k < n_features) folds[(long)blockIdx.y * n_features + f + k] = part[k];
 }
 
+template <bool PARTS>
 static void ztmv_launch(const float* Z, long n_rows, int n, long ldz, const float* th, const float* tl, double* folds,
                         cudaStream_t s) {
   const long nf = zt_folds(n_rows), blocks = (n + kZtCols - 1) / kZtCols;
   const long want = std::max<long>(16L * sm_count() / blocks, 1);   // CTAs per feature block
-  const int per = (int)((nf + want - 1) / want);
+  const int per = PARTS ? kPartFolds : (int)((nf + want - 1) / want);
+  const bool vec = n % 4 == 0 && ldz % 4 == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
   const dim3 grid((unsigned)blocks, (unsigned)((nf + per - 1) / per));
-  if (n % 4 == 0 && ldz % 4 == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0)
-    ztmv_folds_kernel<true><<<grid, kZtThreads, 0, s>>>(Z, n_rows, n, ldz, th, tl, per, folds);
-  else
-    ztmv_folds_kernel<false><<<grid, kZtThreads, 0, s>>>(Z, n_rows, n, ldz, th, tl, per, folds);
+  if (vec) ztmv_folds_kernel<true, PARTS><<<grid, kZtThreads, 0, s>>>(Z, n_rows, n, ldz, th, tl, per, folds);
+  else ztmv_folds_kernel<false, PARTS><<<grid, kZtThreads, 0, s>>>(Z, n_rows, n, ldz, th, tl, per, folds);
 }
 
 // (p and q may be the same vector: each thread reads p[f] before it writes q[f])
-// A CTA adds the folds of 32 features: eight parts of kPartFolds folds at a time
-// (warp g the g-th), then the parts' sums in order.
+// A CTA adds the folds of 32 features: eight parts of F folds at a time (warp g the
+// g-th; F = kPartFolds, or 1 where a part's sum is given), then the parts' sums in order.
+template <int F>
 __global__ void __launch_bounds__(256)
 ztmv_finish_kernel(const double* __restrict__ folds, int n_folds, int n, const double* p, double lambda, double* q) {
   __shared__ double red[8][32];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, f = blockIdx.x * 32 + lane;
   double sum = 0.0;
-  for (int k0 = 0; k0 < n_folds; k0 += 8 * kPartFolds) {
-    const int a = k0 + g * kPartFolds, b = min(a + kPartFolds, n_folds);
-    double v[kPartFolds], acc = 0.0;   // all loads in flight, then the sum in order
+  for (int k0 = 0; k0 < n_folds; k0 += 8 * F) {
+    const int a = k0 + g * F, b = min(a + F, n_folds);
+    double v[F], acc = 0.0;   // all loads in flight, then the sum in order
 #pragma unroll
-    for (int k = 0; k < kPartFolds; ++k) v[k] = f < n && a + k < b ? __ldg(folds + (long)(a + k) * n + f) : 0.0;
+    for (int k = 0; k < F; ++k) v[k] = f < n && a + k < b ? __ldg(folds + (long)(a + k) * n + f) : 0.0;
 #pragma unroll
-    for (int k = 0; k < kPartFolds; ++k)
+    for (int k = 0; k < F; ++k)
       if (a + k < b) acc += v[k];
     red[g][lane] = acc;
     __syncthreads();
     if (g == 0)
-      for (int w = 0; w < 8 && k0 + w * kPartFolds < n_folds; ++w) sum += red[w][lane];
+      for (int w = 0; w < 8 && k0 + w * F < n_folds; ++w) sum += red[w][lane];
     __syncthreads();
   }
   if (g == 0 && f < n) q[f] = sum + lambda * p[f];
@@ -1581,8 +1594,9 @@ struct SolveCtx {
   double lambda;
   double* L;
   long ldl;
-  double* part;  // [folds][n] sums of Z^T t per fold of rows
-  int folds;
+  double* part;  // [sums][n] sums of Z^T t per fold of rows, or per part of kPartFolds folds
+  int sums;
+  bool parts;
   double* t;     // [n_rows]
   float *th, *tl;  // float pair of t (or of y) [n_rows]
   float *ph, *pl;  // float pair of the operand [n]
@@ -1822,6 +1836,21 @@ static int diag_inverses(const double* L, long ldl, int n, double* Dinv, cudaStr
   return QMLR_OK;
 }
 
+// q = Z^T (th + tl) + lambda p
+static int apply_transposed(const SolveCtx& c, const double* p, double lambda, double* q) {
+  if (c.n_rows > 0) {
+    if (c.parts) ztmv_launch<true>(c.Z, c.n_rows, c.n, c.ldz, c.th, c.tl, c.part, c.s);
+    else ztmv_launch<false>(c.Z, c.n_rows, c.n, c.ldz, c.th, c.tl, c.part, c.s);
+    QMLR_LAUNCH_CHECK();
+  } else {
+    QMLR_CUDA_TRY(cudaMemsetAsync(c.part, 0, sizeof(double) * c.n, c.s));
+  }
+  if (c.parts) ztmv_finish_kernel<1><<<(c.n + 31) / 32, 256, 0, c.s>>>(c.part, c.sums, c.n, p, lambda, q);
+  else ztmv_finish_kernel<kPartFolds><<<(c.n + 31) / 32, 256, 0, c.s>>>(c.part, c.sums, c.n, p, lambda, q);
+  QMLR_LAUNCH_CHECK();
+  return QMLR_OK;
+}
+
 // (split: the float pair of p stands in c.ph, c.pl already)
 static int apply_exact(const SolveCtx& c, const double* p, double* q, bool split = false) {
   const long threads = (c.n_rows + kZmvRows - 1) / kZmvRows * 32;
@@ -1839,34 +1868,30 @@ static int apply_exact(const SolveCtx& c, const double* p, double* q, bool split
       zmv_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c.s>>>(c.Z, c.n_rows, c.n, c.ldz, c.ph, c.pl,
                                                                      c.t, c.th, c.tl);
     QMLR_LAUNCH_CHECK();
-    ztmv_launch(c.Z, c.n_rows, c.n, c.ldz, c.th, c.tl, c.part, c.s);
-    QMLR_LAUNCH_CHECK();
-  } else {
-    QMLR_CUDA_TRY(cudaMemsetAsync(c.part, 0, sizeof(double) * c.n, c.s));
   }
-  ztmv_finish_kernel<<<(c.n + 31) / 32, 256, 0, c.s>>>(c.part, c.n_rows > 0 ? c.folds : 1, c.n,
-                                                        p, c.lambda, q);
-  QMLR_LAUNCH_CHECK();
-  return QMLR_OK;
+  return apply_transposed(c, p, c.lambda, q);
 }
 
 }  // namespace qmlr
 
 using namespace qmlr;
 
-extern "C" int64_t qmlr_solve_workspace_bytes(int64_t n_rows, int32_t n_features) {
+static int64_t solve_bytes(int64_t n_rows, int32_t n_features, int64_t sums) {
   const int64_t n = n_features;
-  const int64_t folds = zt_folds(n_rows);
   const int64_t nblk = (n + NB - 1) / NB;
   return n * n * 8                 // factor L
          + nblk * NB * NB * 8      // inverses of the diagonal blocks
          + n * 8                   // triangular-solve scratch
-         + folds * n * 8           // sums of Z^T t per fold of rows
+         + sums * n * 8            // sums of Z^T t per fold (or part) of rows
          + std::max<int64_t>(n_rows, 1) * 16  // t = Z p and its float pair
          + n * 8                   // float pair of the operand
          + 7 * n * 8               // c, r, z, p, q, tmp, published float pairs of the sweeps
          + (int64_t)tc_parts_elems((int)n) * 4   // two split panels of the mixed-precision factor
          + 8 * 8 + 8192;           // scalars + alignment
+}
+
+extern "C" int64_t qmlr_solve_workspace_bytes(int64_t n_rows, int32_t n_features) {
+  return solve_bytes(n_rows, n_features, zt_folds(n_rows));
 }
 
 extern "C" int qmlr_cholesky(double* L, int64_t ldl, int32_t n, int32_t* host_info, void* stream) {
@@ -1931,10 +1956,13 @@ static void carve(char*& p, void** out, size_t bytes) {
   p += (bytes + 255) & ~size_t(255);
 }
 
-extern "C" int64_t qmlr_normal_apply_workspace_bytes(int64_t n_rows, int32_t n_features) {
+static int64_t apply_bytes(int64_t n_rows, int32_t n_features, int64_t sums) {
   const int64_t n = n_features;
-  const int64_t folds = zt_folds(n_rows);
-  return folds * n * 8 + std::max<int64_t>(n_rows, 1) * 16 + n * 8 + 4 * 256;
+  return sums * n * 8 + std::max<int64_t>(n_rows, 1) * 16 + n * 8 + 4 * 256;
+}
+
+extern "C" int64_t qmlr_normal_apply_workspace_bytes(int64_t n_rows, int32_t n_features) {
+  return apply_bytes(n_rows, n_features, zt_folds(n_rows));
 }
 
 extern "C" int qmlr_normal_apply(const float* Z, int64_t n_rows, int32_t n_features, int64_t ldz, double lambda,
@@ -1942,8 +1970,7 @@ extern "C" int qmlr_normal_apply(const float* Z, int64_t n_rows, int32_t n_featu
   QMLR_REQUIRE(p && q, "NULL pointer argument");
   QMLR_REQUIRE(n_features >= 1 && n_rows >= 0 && ldz >= n_features, "bad shapes");
   QMLR_REQUIRE(n_rows == 0 || Z, "Z is NULL");
-  QMLR_REQUIRE(work && work_bytes >= qmlr_normal_apply_workspace_bytes(n_rows, n_features),
-               "workspace too small");
+  QMLR_REQUIRE(work && work_bytes >= apply_bytes(n_rows, n_features, zt_parts(n_rows)), "workspace too small");
   SolveCtx c{};
   c.n = n_features;
   c.n_rows = n_rows;
@@ -1951,10 +1978,11 @@ extern "C" int qmlr_normal_apply(const float* Z, int64_t n_rows, int32_t n_featu
   c.Z = Z;
   c.lambda = lambda;
   c.s = as_stream(stream);
-  c.folds = (int)zt_folds(n_rows);
+  c.parts = work_bytes < qmlr_normal_apply_workspace_bytes(n_rows, n_features);
+  c.sums = (int)(c.parts ? zt_parts(n_rows) : zt_folds(n_rows));
   char* w = static_cast<char*>(work);
   void *vpart, *vt, *vth, *vph;
-  carve(w, &vpart, (size_t)c.folds * c.n * 8);
+  carve(w, &vpart, (size_t)c.sums * c.n * 8);
   carve(w, &vt, (size_t)std::max<int64_t>(n_rows, 1) * 8);
   carve(w, &vth, (size_t)std::max<int64_t>(n_rows, 1) * 8);
   carve(w, &vph, (size_t)c.n * 8);
@@ -1975,8 +2003,7 @@ extern "C" int qmlr_gram_solve(const float* G, const float* Z, int64_t n_rows, i
   QMLR_REQUIRE(n_rows == 0 || (Z && y), "Z/y are NULL");
   QMLR_REQUIRE(lambda >= 0, "lambda must be >= 0");
   QMLR_REQUIRE(opts->max_iter >= 0, "max_iter must be >= 0");
-  QMLR_REQUIRE(work && work_bytes >= qmlr_solve_workspace_bytes(n_rows, n_features),
-               "workspace too small");
+  QMLR_REQUIRE(work && work_bytes >= solve_bytes(n_rows, n_features, zt_parts(n_rows)), "workspace too small");
   QMLR_REQUIRE(opts->method == QMLR_SOLVE_PCG || opts->method == QMLR_SOLVE_REFINE,
                "unknown solve method %d", opts->method);
   QMLR_REQUIRE(opts->factor == QMLR_FACTOR_FP64 || opts->factor == QMLR_FACTOR_MIXED,
@@ -1991,14 +2018,15 @@ extern "C" int qmlr_gram_solve(const float* G, const float* Z, int64_t n_rows, i
   c.lambda = lambda;
   c.ldl = n;
   c.s = s;
-  c.folds = (int)zt_folds(n_rows);
+  c.parts = work_bytes < qmlr_solve_workspace_bytes(n_rows, n_features);
+  c.sums = (int)(c.parts ? zt_parts(n_rows) : zt_folds(n_rows));
   char* p = static_cast<char*>(work);
   void *vL, *vpart, *vt, *vc, *vr, *vz, *vp, *vq, *vtmp, *vsc, *vdinv, *vtri, *vsplit, *vth, *vph, *vpub;
   const int nblk = (n + NB - 1) / NB;
   carve(p, &vL, (size_t)n * n * 8);
   carve(p, &vdinv, (size_t)nblk * NB * NB * 8);
   carve(p, &vtri, (size_t)n * 8);
-  carve(p, &vpart, (size_t)c.folds * n * 8);
+  carve(p, &vpart, (size_t)c.sums * n * 8);
   carve(p, &vt, (size_t)std::max<int64_t>(n_rows, 1) * 8);
   carve(p, &vc, (size_t)n * 8);
   carve(p, &vr, (size_t)n * 8);
@@ -2030,10 +2058,8 @@ extern "C" int qmlr_gram_solve(const float* G, const float* Z, int64_t n_rows, i
   if (n_rows > 0) {
     split_kernel<<<(unsigned)((n_rows + 255) / 256), 256, 0, s>>>(n_rows, y, c.th, c.tl);
     QMLR_LAUNCH_CHECK();
-    ztmv_launch(Z, n_rows, n, ldz, c.th, c.tl, c.part, s);
-    QMLR_LAUNCH_CHECK();
-    ztmv_finish_kernel<<<(n + 31) / 32, 256, 0, s>>>(c.part, c.folds, n, cv, 0.0, cv);
-    QMLR_LAUNCH_CHECK();
+    const int rc = apply_transposed(c, cv, 0.0, cv);
+    if (rc) return rc;
   } else {
     QMLR_CUDA_TRY(cudaMemsetAsync(cv, 0, sizeof(double) * n, s));
   }
