@@ -929,12 +929,12 @@ template <bool DF>
 __global__ void __launch_bounds__(256)
 fwd_flow_kernel(const double* __restrict__ L, long ldl, const double* __restrict__ Dinv, int n,
                 const double* __restrict__ r, double* __restrict__ y, double* yp, int* err) {
-  __shared__ double rb[2][NB];   // (by turns: a warp may be a block ahead)
-  __shared__ int fail;
+  __shared__ double rb[2][NB];   // by turns, and so is the flag: a warp may be a block ahead, and
+  __shared__ int fail[2];        // one that gives up there must not end a warp in this block
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rs = 4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1);
   const int nblk = (n + NB - 1) / NB;
-  if (tid == 0) fail = 0;
+  if (tid < 2) fail[tid] = 0;
   __syncthreads();
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
     const int r0 = b * NB, nb = min(NB, n - r0);
@@ -994,7 +994,8 @@ fwd_flow_kernel(const double* __restrict__ L, long ldl, const double* __restrict
       }
       if (!(ok = consume(j + 2, T2, X2))) break;
     }
-    if (!ok) fail = 1;
+    const int turn = (b / gridDim.x) & 1;
+    if (!ok) fail[turn] = 1;
     // reduce-scatter of the 8 row sums over the warp's lanes
     {
       const bool h = lane & 16;
@@ -1022,10 +1023,10 @@ fwd_flow_kernel(const double* __restrict__ L, long ldl, const double* __restrict
     }
     acc[0].add(acc[0].xor_lane(2));
     acc[0].add(acc[0].xor_lane(1));
-    double* rs64 = rb[(b / gridDim.x) & 1];
+    double* rs64 = rb[turn];
     if ((lane & 3) == 0) rs64[myrow] = myrow < nb ? rhs_minus<DF>(rv, rp, acc[0]) : 0.0;
     __syncthreads();
-    if (fail) return;
+    if (fail[turn]) return;
     double v;
     if constexpr (DF) v = block_matvec_pairs(dv, rs64);
     else v = block_matvec_reg(dv, rs64);
