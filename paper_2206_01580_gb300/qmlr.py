@@ -950,15 +950,30 @@ def force_rows(tangents, jac_ptr, mol_ptr, sin_t, sign_bits, T: int, n_features:
     return out
 
 
+def _check_rows(out, row0: int, n_rows: int, nf: int):
+    """out is a device matrix of float32 rows that holds n_rows rows of nf columns from row row0."""
+    assert out.dtype == torch.float32 and out.dim() == 2 and out.stride(1) == 1, "out must be float32 rows"
+    assert out.shape[1] >= nf and out.stride(0) >= nf, "out has too few columns"
+    assert row0 >= 0 and out.shape[0] >= row0 + n_rows, "out has too few rows"
+    assert out.is_cuda, "out must be on the device"
+
+
 def force_rows_tc(tangents, jac_ptr, mol_ptr, sin_t, tables, T: int, sigma: float, out=None, row0: int = 0):
     """Force rows (as force_rows) from the tensor-core chains; sin_t [N_F / 128, n_atoms, 128]
     from sorf_segment_sum_tc."""
+    assert sin_t.dtype == torch.float32 and sin_t.dim() == 3 and sin_t.shape[2] == 128 and sin_t.is_contiguous()
+    n_atoms, nf = sin_t.shape[1], sin_t.shape[0] * sin_t.shape[2]
+    if out is not None:
+        _check_rows(out, row0, 3 * n_atoms, nf)
+    assert out is not None or row0 == 0, "row0 needs an out"
+    assert sin_t.is_cuda and tables.is_cuda and tables.is_contiguous()
+    assert tables.numel() * tables.element_size() >= lib().qmlr_sorf_tc_table_bytes(nf), "tables of fewer features"
     tangents = _dev(tangents, torch.float32)
     mol_ptr = _dev(mol_ptr, torch.int32)
+    jac_ptr = _dev(jac_ptr, torch.int64)
     n_mol = mol_ptr.shape[0] - 1
-    n_atoms, nf = sin_t.shape[1], sin_t.shape[0] * sin_t.shape[2]
+    assert jac_ptr.shape == (n_mol + 1,)
     n_rows, d = tangents.shape
-    assert sin_t.dtype == torch.float32 and sin_t.is_contiguous()
     if out is None:
         out = torch.empty((3 * n_atoms, nf), device="cuda", dtype=torch.float32)
     wb = lib().qmlr_force_rows_tc_workspace_bytes(n_rows)
