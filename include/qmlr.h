@@ -476,8 +476,10 @@ int qmlr_sorf_segment_sum_sin_tc(const float* x, int32_t d, const int32_t* mol_p
  *               aligned (FP16 parts and scales of the tangents, triple indices)
  * Errors: QMLR_EINVAL for d != 128, T > 3, N_F not a multiple of 128, NULL or
  * misaligned pointers (tangents, tables: 16 bytes), a workspace below the
- * required size, more than ~1.07e9 Jacobian rows. Asynchronous on `stream`;
- * deterministic; allocates nothing; every wait is bounded (device error 4).
+ * required size, Jacobian rows without atoms, more than ~1.006e9 Jacobian rows.
+ * Rows of a molecule whose entries of mol_ptr and jac_ptr do not match each other,
+ * n_atoms or n_jac_rows are left as they are (device error 3). Asynchronous on
+ * `stream`; deterministic; allocates nothing; every wait is bounded (device error 4).
  */
 int64_t qmlr_force_rows_tc_workspace_bytes(int64_t n_jac_rows);
 int qmlr_force_rows_tc(const float* tangents, int32_t d, const int64_t* jac_ptr, int64_t n_jac_rows,
