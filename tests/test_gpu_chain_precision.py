@@ -61,3 +61,19 @@ def test_truncations_leave_no_bias(q, sizes, T, sigma):
     t = (np.random.default_rng(2).normal(size=(N, D)) * SIZES[sizes]).astype(np.float32)
     (bias, _), _ = _errors(q, t, T, sigma)
     assert abs(bias) <= 2.0e-8, bias
+
+
+@pytest.mark.parametrize("power", [-100, 85, 100, 115])
+def test_rows_of_any_size(q, power):
+    """Vectors times a power of two give the rows times it, bit for bit: the largest of N x D normal values is below
+    2^3, so |t| < 2^7 and |W t| <= sqrt(D) / sigma |t| < 2^10 at power 0, finite at 2^115."""
+    signs, _ = synth.sorf_draw(np.random.default_rng(0), NF, D, 3)
+    t = np.random.default_rng(3).normal(size=(N, D)).astype(np.float32)
+    n = N // 3
+    ptr = torch.arange(n + 1, dtype=torch.int32, device="cuda")
+    args = (3 * ptr.long(), ptr, torch.ones((NF // D, n, D), device="cuda"),
+            q.sorf_tc_tables(q.pack_signs(signs), 3, NF), 3, 2.0)
+    want = q.force_rows_tc(t, *args)
+    got = q.force_rows_tc(np.ldexp(t, power).astype(np.float32), *args)
+    assert bool(torch.isfinite(got).all()) and torch.equal(got, torch.ldexp(want, torch.tensor(power, device="cuda")))
+    assert q.device_status() == 0
