@@ -389,9 +389,7 @@ int32_t qmlr_sorf_parts(int32_t n_features, int32_t d);
  *   gx          float [n_part][n_atoms][d]  dE/dx_I from the stacks of part p, or NULL
  *                                          (energies only)
  * n_part = qmlr_sorf_parts(n_features, d); qmlr_project_t sums the parts.
- * Takes 2 N_F floats of stream-ordered scratch for large batches (a copy of b and
- * alpha with the stacks contiguous); under stream capture, or where there is no
- * memory for it, it reads them in place, with the same results.
+ * Allocates nothing.
  */
 int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr, int32_t n_mol,
                    int32_t n_atoms, const uint32_t* sign_bits, int32_t T, const float* b,

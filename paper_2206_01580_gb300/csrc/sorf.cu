@@ -17,6 +17,8 @@
 // CTA's stacks in shared memory.
 #include "sorf_math.cuh"
 
+#include <type_traits>
+
 namespace qmlr {
 
 constexpr int kStacksPerCta = 128;
@@ -239,14 +241,12 @@ sorf_mol_kernel(SorfArgs a) {
   for (int f = tid; f < nf; f += nt) o[f] = a.pref * acc[(f / D) * LD + f % D];
 }
 
-// bT[i * n_stack + s] = b[s * d + i], and the same for alpha when it is given
-__global__ void transpose_phases_kernel(const float* __restrict__ b, const float* __restrict__ alpha, int d, int n_stack,
-                                        float* __restrict__ bT, float* __restrict__ alphaT) {
+// bT[i * n_stack + s] = b[s * d + i]
+__global__ void transpose_phases_kernel(const float* __restrict__ b, int d, int n_stack, float* __restrict__ bT) {
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d * n_stack) return;
   const int s = f / d, i = f % d;
   bT[(long)i * n_stack + s] = b[f];
-  if (alpha) alphaT[(long)i * n_stack + s] = alpha[f];
 }
 
 // ---------------------------------------------------------------------------
@@ -339,9 +339,30 @@ __device__ __forceinline__ void reduce_scatter_step(float (&v)[D], int lane) {
 
 // The chains, phases and products run on packed pairs (half the instructions of
 // the scalar form, which missed the instruction cache: 1.2 of 3.0 stall cycles
-// per issue at D = 128), and the phases and weights are read at a uniform row
-// address plus the stack's offset (MINOR: stack-minor order, coalesced; else the
-// natural order). 53 k atoms at N_F = 16384, energies only: 1.39 -> 1.13 ms.
+// per issue at D = 128). 53 k atoms at N_F = 16384, energies only: 1.39 -> 1.13 ms.
+// MINOR: the phases and weights lie stack-minor and are read at a uniform row address
+// plus the stack (the model's copies). Else they lie in natural order, where a stack's
+// values are contiguous: a warp copies the 32 x 32 block of its stacks and the next
+// dimensions into shared memory while it works on the one before, and each lane reads
+// its stack's row. E + F of 20 000 atoms at N_F = 16384: 5.8 ms read directly, where
+// each load touches 32 lines, 0.90 so, 0.87 from a stack-minor copy; but memory for
+// that copy in every call cost the host ~150 us after each synchronisation, when the
+// stream-ordered pool has given its memory back.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+template <int D>
+__host__ __device__ constexpr int stage_dims() { return D < 32 ? D : 32; }
+// floats per row of a block: 16-byte reads of eight consecutive rows fall into different banks
+template <int D>
+__host__ __device__ constexpr int stage_ld() { return stage_dims<D>() + 4; }
+// bytes of a warp's blocks: two in turn of phases and weights
+template <int D>
+__host__ __device__ constexpr int stage_bytes() { return 2 * 2 * 32 * stage_ld<D>() * 4; }
+
 template <int D, bool GRAD, bool MINOR>
 __global__ void __launch_bounds__(kStacksPerCta, GRAD ? 2 : 3)
 sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
@@ -351,7 +372,8 @@ sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
   float* xs = smem;                                           // [D]
   double* red = reinterpret_cast<double*>(smem + D + 4);      // [NW]
   uint32_t* sg = reinterpret_cast<uint32_t*>(red + NW);       // [T*W][nt]
-  float* work = reinterpret_cast<float*>(sg + 4 * W * kStacksPerCta);  // gradient partials
+  float* work = reinterpret_cast<float*>(sg + 4 * W * blockDim.x);  // gradient partials
+  constexpr int kWork = GRAD ? (D >= 32 ? NW * D : kStacksPerCta * (D + 1)) : 0;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int atom = blockIdx.x, part = blockIdx.y;
   const int s = part * kStacksPerCta + tid;
@@ -360,6 +382,29 @@ sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
   for (int k = 0; k < a.T * W; ++k) sg[k * nt + tid] = active ? __ldg(a.sign_bits + (long)s * a.T * W + k) : 0u;
   __syncthreads();
   if (tid < 32 && part == 0) check_range<D>(xs, a.x2max, tid, a.err);
+  // natural order: phases and weights of the warp's stacks, dimensions c CH .. + CH - 1
+  constexpr int CH = stage_dims<D>(), LD = stage_ld<D>();
+  [[maybe_unused]] float* blocks = work + kWork + warp * (stage_bytes<D>() / 4);
+  [[maybe_unused]] auto fetch = [&](int c) {
+    float* dst = blocks + (c & 1) * 2 * 32 * LD;
+    const int s0 = part * kStacksPerCta + warp * 32, rows = min(32, a.n_stack - s0);
+    const long src = (long)s0 * D + c * CH;
+    auto copy = [&](auto width) {   // `width` floats at a time
+      constexpr int V = decltype(width)::value;
+#pragma unroll 8
+      for (int u = lane; u < 32 * CH / V; u += 32) {
+        const int r = u / (CH / V), k = u % (CH / V) * V;
+        if (r >= rows) break;
+        copy_async<4 * V>(dst + r * LD + k, a.b + src + r * D + k);
+        copy_async<4 * V>(dst + (32 + r) * LD + k, a.alpha + src + r * D + k);
+      }
+    };
+    if (((reinterpret_cast<uintptr_t>(a.b) | reinterpret_cast<uintptr_t>(a.alpha)) & 15) == 0)
+      copy(std::integral_constant<int, 4>());
+    else copy(std::integral_constant<int, 1>());
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if constexpr (!MINOR) fetch(0);
   f32x2 v[D / 2];
 #pragma unroll
   for (int i = 0; i < D / 2; ++i) v[i] = pack2(xs[2 * i], xs[2 * i + 1]);
@@ -371,25 +416,49 @@ sorf_atom_kernel(SorfArgs a, double* __restrict__ atom_e) {
     fwht2<D>(v);
   }
   float e = 0.f;
-  if (active) {
-    const f32x2 scale = pack2(a.scale, a.scale);
-    const float gs = -a.pref * a.scale;
-    const int at = MINOR ? s : s * D;
-    const long step = MINOR ? a.n_stack : 1;
+  const f32x2 scale = pack2(a.scale, a.scale);
+  const float gs = -a.pref * a.scale;
+  auto pair_of = [&](int i, float al0, float al1, float b0, float b1) {   // features i, i + 1 of the stack
+    float r0, r1;
+    unpack2(reduce_phase2(fma2(v[i / 2], scale, pack2(b0, b1))), r0, r1);
+    e = fmaf(al0, __cosf(r0), e);
+    e = fmaf(al1, __cosf(r1), e);
+    if (GRAD) v[i / 2] = mul2(mul2(pack2(gs, gs), pack2(al0, al1)), pack2(__sinf(r0), __sinf(r1)));
+  };
+  if constexpr (MINOR) {
+    if (active) {
 #pragma unroll
-    for (int i = 0; i < D; i += 2) {
-      const float* bi = a.b + i * step;      // uniform
-      const float* ai = a.alpha + i * step;
-      const float al0 = __ldg(ai + at), al1 = __ldg(ai + step + at);
-      float r0, r1;
-      unpack2(reduce_phase2(fma2(v[i / 2], scale, pack2(__ldg(bi + at), __ldg(bi + step + at)))), r0, r1);
-      e = fmaf(al0, __cosf(r0), e);
-      e = fmaf(al1, __cosf(r1), e);
-      if (GRAD) v[i / 2] = mul2(mul2(pack2(gs, gs), pack2(al0, al1)), pack2(__sinf(r0), __sinf(r1)));
+      for (int i = 0; i < D; i += 2) {
+        const float* bi = a.b + (long)i * a.n_stack;      // uniform
+        const float* ai = a.alpha + (long)i * a.n_stack;
+        const float al0 = __ldg(ai + s), al1 = __ldg(ai + a.n_stack + s);
+        pair_of(i, al0, al1, __ldg(bi + s), __ldg(bi + a.n_stack + s));
+      }
     }
-  } else if (GRAD) {
+  } else {
 #pragma unroll
-    for (int i = 0; i < D / 2; ++i) v[i] = pack2(0.f, 0.f);
+    for (int c = 0; c < D / CH; ++c) {
+      if (c + 1 < D / CH) fetch(c + 1);
+      if (c + 1 < D / CH) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+      const float4* bs = reinterpret_cast<const float4*>(blocks + ((c & 1) * 2 * 32 + lane) * LD);
+      const float4* as = bs + 32 * LD / 4;
+#pragma unroll
+      for (int i = 0; i < CH / 4; ++i) {
+        const float4 al = as[i], bb = bs[i];
+        pair_of(c * CH + 4 * i, al.x, al.y, bb.x, bb.y);
+        pair_of(c * CH + 4 * i + 2, al.z, al.w, bb.z, bb.w);
+      }
+      __syncwarp();
+    }
+  }
+  if (!active) {
+    e = 0.f;
+    if (GRAD) {
+#pragma unroll
+      for (int i = 0; i < D / 2; ++i) v[i] = pack2(0.f, 0.f);
+    }
   }
   double ed = (double)e;
 #pragma unroll
@@ -504,8 +573,9 @@ template <int D, bool GRAD, bool MINOR>
 static int launch_atoms(const SorfArgs& a, double* atom_e, int n_mol, double* E, cudaStream_t s) {
   const int nt = std::min(kStacksPerCta, ((a.n_stack + 31) / 32) * 32);
   constexpr int W = (D + 31) / 32;
-  const size_t smem = (size_t)(D + 4) * 4 + (kStacksPerCta / 32) * 8 + (size_t)4 * W * kStacksPerCta * 4 +
-                      (GRAD ? (D >= 32 ? (size_t)(kStacksPerCta / 32) * D * 4 : (size_t)nt * (D + 1) * 4) : 0);
+  const size_t smem = (size_t)(D + 4) * 4 + (kStacksPerCta / 32) * 8 + (size_t)4 * W * nt * 4 +
+                      (GRAD ? (D >= 32 ? (size_t)(kStacksPerCta / 32) * D * 4 : (size_t)kStacksPerCta * (D + 1) * 4) : 0) +
+                      (MINOR ? 0 : (size_t)(nt / 32) * stage_bytes<D>());
   QMLR_CUDA_TRY(smem_attr_once((const void*)sorf_atom_kernel<D, GRAD, MINOR>, 227 * 1024));
   if (a.n_atoms > 0) {
     dim3 grid(a.n_atoms, a.n_part);
@@ -587,7 +657,7 @@ static int launch_mol(const SorfArgs& a0, int n_mol, cudaStream_t s) {
   const int nf = a0.n_stack * D;
   float* bT = nullptr;
   QMLR_CUDA_TRY(cudaMallocAsync(&bT, sizeof(float) * nf, s));
-  transpose_phases_kernel<<<(nf + 255) / 256, 256, 0, s>>>(a0.b, nullptr, D, a0.n_stack, bT, nullptr);
+  transpose_phases_kernel<<<(nf + 255) / 256, 256, 0, s>>>(a0.b, D, a0.n_stack, bT);
   int rc = QMLR_OK;
   {
     cudaError_t e = cudaGetLastError();
@@ -735,9 +805,6 @@ extern "C" int qmlr_force_rows(const float* tangents, int32_t d, const int64_t* 
   }
 }
 
-// Atoms up to which qmlr_sorf_grad reads b and alpha in place.
-static constexpr int kSorfNaturalAtoms = 128;
-
 extern "C" int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr, int32_t n_mol,
                               int32_t n_atoms, const uint32_t* sign_bits, int32_t T, const float* b,
                               int32_t n_features, double sigma, const float* alpha, double* atom_energy,
@@ -750,38 +817,6 @@ extern "C" int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr,
   if (n_mol == 0) return QMLR_OK;
   QMLR_REQUIRE(mol_ptr && energies && atom_energy, "NULL pointer argument");
   QMLR_REQUIRE(n_atoms == 0 || (x && sign_bits && b && alpha), "NULL pointer argument");
-  // Phases and weights in stack-minor order (stream-ordered scratch) for coalesced
-  // loads: in natural order each load touches 32 lines, 422 us of E + F for a
-  // 3000-atom periodic cell at N_F = 16384. Natural order where the scratch and its
-  // launch cost more than the loads (a call of up to 128 atoms 27-33 us at 512 to 16384
-  // features, with the scratch 33-36; from 150 atoms on the scratch wins), under
-  // capture (a graph that owns memory has fewer uses), and when there is no memory for
-  // it; the results have the same bits.
-  cudaStream_t st = as_stream(stream);
-  float* bT = nullptr;
-  if (n_atoms > kSorfNaturalAtoms) {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
-        cudaMallocAsync(&bT, sizeof(float) * 2 * (size_t)n_features, st) != cudaSuccess) {
-      bT = nullptr;
-      cudaGetLastError();
-    }
-  }
-  if (bT == nullptr) {
-    const SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, b, n_features, sigma, alpha, gx);
-    return sorf_energy_atoms<false>(a, d, atom_energy, n_mol, energies, gx != nullptr, st);
-  }
-  transpose_phases_kernel<<<(n_features + 255) / 256, 256, 0, st>>>(b, alpha, d, n_features / d, bT, bT + n_features);
-  count_launch();
-  int rc = QMLR_OK;
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    set_error("kernel launch failed: %s", cudaGetErrorString(e));
-    rc = QMLR_ECUDA;
-  } else {
-    const SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, bT, n_features, sigma, bT + n_features, gx);
-    rc = sorf_energy_atoms<true>(a, d, atom_energy, n_mol, energies, gx != nullptr, st);
-  }
-  cudaFreeAsync(bT, st);
-  return rc;
+  const SorfArgs a = make_sorf_args(x, d, mol_ptr, n_atoms, sign_bits, T, b, n_features, sigma, alpha, gx);
+  return sorf_energy_atoms<false>(a, d, atom_energy, n_mol, energies, gx != nullptr, as_stream(stream));
 }
