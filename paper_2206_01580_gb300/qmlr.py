@@ -185,7 +185,10 @@ def _ptr(t):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of the current device's current stream (without the Stream object around it, which costs 3 us a call)."""
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
 
 
 def _dev(t, dtype):
