@@ -1811,11 +1811,11 @@ __global__ void __launch_bounds__(32 * kWarpsFwd, 6)
 fchl19_periodic_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem, int n_atoms, Cell9 cell,
                        const int64_t* __restrict__ env_ptr, const int32_t* __restrict__ env_atom,
                        const int32_t* __restrict__ env_shift, int max_env, int envp, Fchl19Consts c,
-                       float* __restrict__ rep, int rep_ld, int* err) {
+                       float* __restrict__ rep, int rep_ld, long wide_from, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarpsFwd + warp;
-  if (i >= n_atoms) return;
+  if (i >= n_atoms || __ldg(env_ptr + n_atoms) >= wide_from) return;
   const RegWarp s = carve_reg(smem_raw + warp * reg_warp_bytes(envp), envp);
   const BinConsts kb = bin_consts(c, lane);
   float* out = rep + (size_t)i * rep_ld;
@@ -1853,14 +1853,14 @@ fchl19_periodic_vjp_kernel(const float* __restrict__ coords, const int32_t* __re
                            Cell9 cell, const int64_t* __restrict__ env_ptr, const int32_t* __restrict__ env_atom,
                            const int32_t* __restrict__ env_shift, int max_env, int envp, Fchl19Consts c,
                            const float* __restrict__ grad_rep, int rep_ld, float* __restrict__ contrib,
-                           int* err) {
+                           long wide_from, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarpsVjp + warp;
-  if (i >= n_atoms) return;
+  const long E = __ldg(env_ptr + n_atoms);
+  if (i >= n_atoms || E >= wide_from) return;
   const int rp = (c.rep_dim + 3) & ~3;
   VjpWarp s = carve_vjp(smem_raw + warp * vjp_warp_bytes(envp + 4, rp), envp + 4, rp);
-  const long E = __ldg(env_ptr + n_atoms);
   const long e0 = __ldg(env_ptr + i), e1 = __ldg(env_ptr + i + 1);
   const int ne = (int)(e1 - e0);
   if (e1 - e0 > max_env || e1 < e0) {
@@ -1946,19 +1946,13 @@ __global__ void __launch_bounds__(32 * kWideWarps)
 fchl19_periodic_wide_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem, int n_atoms, Cell9 cell,
                             const int64_t* __restrict__ env_ptr, const int32_t* __restrict__ env_atom,
                             const int32_t* __restrict__ env_shift, int max_env, int envp, Fchl19Consts c,
-                            float* __restrict__ rep, int rep_ld, int* err) {
+                            float* __restrict__ rep, int rep_ld, long wide_from, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
   __shared__ int counts[kWideWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x;
+  if (__ldg(env_ptr + n_atoms) < wide_from) return;
   const BinConsts kb = bin_consts(c, lane);
   const int rows3 = 2 * kb.np * c.n3;
-  float* out = rep + (size_t)i * rep_ld;
-  const long e0 = __ldg(env_ptr + i), e1 = __ldg(env_ptr + i + 1);
-  if (e1 - e0 > max_env || e1 < e0) {
-    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
-    for (int k = threadIdx.x; k < rep_ld; k += blockDim.x) out[k] = 0.0f;
-    return;
-  }
   RegWarp s;
   s.nb_u = reinterpret_cast<float4*>(smem_raw);
   s.nb_2b = s.nb_u + envp;
@@ -1967,6 +1961,13 @@ fchl19_periodic_wide_kernel(const float* __restrict__ coords, const int32_t* __r
   float* sums = reinterpret_cast<float*>(s.nb_2b + envp + (size_t)kWideWarps * (kPairBlock + 4));
   float* row = sums + (size_t)kWideWarps * rows3;
   s.nb_el = reinterpret_cast<int*>(row + rows3);
+  float* out = rep + (size_t)i * rep_ld;
+  const long e0 = __ldg(env_ptr + i), e1 = __ldg(env_ptr + i + 1);
+  if (e1 - e0 > max_env || e1 < e0) {
+    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
+    for (int k = threadIdx.x; k < rep_ld; k += blockDim.x) out[k] = 0.0f;
+    return;
+  }
   const int n = periodic_list_wide(coords, elem, n_atoms, cell, env_atom, env_shift, e0, e1, i, c, warp, lane, counts,
                                    err, [&](int slot, float dx, float dy, float dz, float r2, int el, int) {
                                      store_neighbour(s, slot, dx, dy, dz, r2, el, c);
@@ -1979,21 +1980,14 @@ __global__ void __launch_bounds__(32 * kWideWarps)
 fchl19_periodic_vjp_wide_kernel(const float* __restrict__ coords, const int32_t* __restrict__ elem, int n_atoms,
                                 Cell9 cell, const int64_t* __restrict__ env_ptr, const int32_t* __restrict__ env_atom,
                                 const int32_t* __restrict__ env_shift, int max_env, int envp, Fchl19Consts c,
-                                const float* __restrict__ grad_rep, int rep_ld, float* __restrict__ contrib, int* err) {
+                                const float* __restrict__ grad_rep, int rep_ld, float* __restrict__ contrib,
+                                long wide_from, int* err) {
   extern __shared__ __align__(16) char smem_raw[];
   __shared__ int counts[kWideWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x;
   const int rp = (c.rep_dim + 3) & ~3, accs = 3 * (envp + 4);
   const long E = __ldg(env_ptr + n_atoms);
-  const long e0 = __ldg(env_ptr + i), e1 = __ldg(env_ptr + i + 1);
-  const int ne = (int)(e1 - e0);
-  if (e1 - e0 > max_env || e1 < e0) {
-    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
-    if (e1 >= e0)
-      for (long k = 3 * e0 + threadIdx.x; k < 3 * e1; k += blockDim.x) contrib[k] = 0.0f;
-    if (threadIdx.x < 3) contrib[3 * (E + i) + threadIdx.x] = 0.0f;
-    return;
-  }
+  if (E < wide_from) return;
   VjpWarp s;
   s.stage = nullptr;
   s.nb_u = reinterpret_cast<float4*>(smem_raw);
@@ -2003,6 +1997,15 @@ fchl19_periodic_vjp_wide_kernel(const float* __restrict__ coords, const int32_t*
   s.nb_idx = s.nb_el + envp;
   float* facc = reinterpret_cast<float*>(s.nb_idx + envp);   // [kWideWarps][accs]
   s.facc = facc + (size_t)warp * accs;
+  const long e0 = __ldg(env_ptr + i), e1 = __ldg(env_ptr + i + 1);
+  const int ne = (int)(e1 - e0);
+  if (e1 - e0 > max_env || e1 < e0) {
+    if (threadIdx.x == 0) record_device_error(err, DEV_MOL_TOO_LARGE);
+    if (e1 >= e0)
+      for (long k = 3 * e0 + threadIdx.x; k < 3 * e1; k += blockDim.x) contrib[k] = 0.0f;
+    if (threadIdx.x < 3) contrib[3 * (E + i) + threadIdx.x] = 0.0f;
+    return;
+  }
   const float* grow = grad_rep + (size_t)i * rep_ld;
   const int sh = c.base3 & 1;   // the layout of load_grad_row
   for (int k = threadIdx.x; k < c.rep_dim; k += blockDim.x) s.g[k + (k >= c.base3 ? sh : 0)] = __ldg(grow + k);
@@ -2055,13 +2058,33 @@ __global__ void periodic_reduce_kernel(int n_atoms, const int64_t* __restrict__ 
 }
 
 constexpr int kPeriodicWideMax = 224 * 1024;   // dynamic shared memory (the counts are static)
-// Periodic systems whose centres get a CTA each (about 85 entries and 2600-3700
-// pairs per centre): forward 219 -> 48 us and adjoint 272 -> 62 us at 96 atoms,
-// 173 -> 69 and 226 -> 89 at 600, 253 -> 210 and 326 -> 265 at 3000, 810 -> 792
-// and 1111 -> 944 at 12 000; at 16 848 the forward loses 3 %, the adjoint still
-// gains. With fewer than 32 entries a centre has less than two pair blocks.
-static bool wide_periodic(int max_env) { return max_env >= 32; }
-constexpr int kPeriodicWideFwdAtoms = 12288;
+// Periodic systems whose centres get a CTA each: those with enough entries per centre
+// in the mean for their number of atoms. The mean counts, which the device alone
+// knows; max_env is that of the densest place (a system of 12 000 atoms with 22 entries
+// in the mean and 41 at most: forward 96 us by warps, 289 by CTAs). So where max_env
+// leaves it open, both forms are launched, and the kernels of one return at once (about
+// 1 us per 1000 atoms).
+// The lines lie where the two were equal, us by warps / by CTAs: forward 600 atoms with
+// 22 entries in the mean 33 / 31, 1200 with 31 48 / 43, 2000 with 40 74 / 72, 4000 with
+// 50 152 / 144, 8000 with 59 332 / 315, 12 000 with 72 643 / 643; adjoint 4000 with 23
+// 72 / 66, 8000 with 32 157 / 150, 12 000 with 41 305 / 290, 20 000 with 41 473 / 479.
+// With 90 entries: forward 600 atoms 201 / 70, 4000 488 / 311, 12 000 1064 / 877, adjoint
+// 248 / 91, 578 / 378, 1289 / 1035. With fewer than 32 entries at most a centre has less
+// than two pair blocks.
+constexpr int kPeriodicWideFwdAtoms = 12288;   // 16 848 atoms with 85 entries: the forward loses 3 %
+
+// Entries of the whole system from which its centres get a CTA each (0: always), the mean
+// growing by `step` with each doubling of the atoms beyond `base`.
+static long periodic_wide_from(double step, double base, int n_atoms) {
+  const double mean = step * std::log2(n_atoms / base);
+  return mean < 24.0 ? 0 : (long)(mean * n_atoms);
+}
+// Whether a system of at most max_env entries per centre is likely to have that many (the
+// densest centre of a liquid or a framework has 1.3-1.5 times the mean).
+static bool may_be_wide(long wide_from, int max_env, int n_atoms) {
+  return max_env >= 32 && (long)max_env * n_atoms >= wide_from + wide_from / 7;
+}
+constexpr long kNeverWide = 1L << 62;
 
 // Batches whose atoms get a CTA each instead of a warp (forward and adjoint):
 // molecules of 64 atoms or more may occur and the mean says that they do. A
@@ -2309,17 +2332,20 @@ extern "C" int qmlr_fchl19_periodic(const float* coords, const int32_t* elem, in
   const int envp = (std::max(max_env, 1) + 3) & ~3;
   const size_t smem = kWarpsFwd * reg_warp_bytes(envp);
   QMLR_REQUIRE(smem <= 227 * 1024, "max_env too large for shared memory");
-  const size_t wide = periodic_wide_smem(envp, rd - p->n_el * p->n2);
-  if (wide_periodic(max_env) && n_atoms <= kPeriodicWideFwdAtoms && wide <= kPeriodicWideMax) {
+  const long from = periodic_wide_from(12.0, 200.0, n_atoms);
+  const bool wide = n_atoms <= kPeriodicWideFwdAtoms && may_be_wide(from, max_env, n_atoms);
+  if (wide) {   // (less shared memory than required above)
     QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_periodic_wide_kernel, kPeriodicWideMax));
-    fchl19_periodic_wide_kernel<<<n_atoms, 32 * kWideWarps, wide, as_stream(stream)>>>(
-        coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, rep, rep_ld, device_error_ptr());
+    fchl19_periodic_wide_kernel<<<n_atoms, 32 * kWideWarps, periodic_wide_smem(envp, rd - p->n_el * p->n2),
+                                  as_stream(stream)>>>(coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift,
+                                                       max_env, envp, c, rep, rep_ld, from, device_error_ptr());
     QMLR_LAUNCH_CHECK();
-    return QMLR_OK;
+    if (from == 0) return QMLR_OK;
   }
   QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_periodic_kernel, 227 * 1024));
   fchl19_periodic_kernel<<<(n_atoms + kWarpsFwd - 1) / kWarpsFwd, 32 * kWarpsFwd, smem, as_stream(stream)>>>(
-      coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, rep, rep_ld, device_error_ptr());
+      coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, rep, rep_ld,
+      wide ? from : kNeverWide, device_error_ptr());
   QMLR_LAUNCH_CHECK();
   return QMLR_OK;
 }
@@ -2344,19 +2370,22 @@ extern "C" int qmlr_fchl19_periodic_vjp(const float* coords, const int32_t* elem
   const size_t smem = kWarpsVjp * vjp_warp_bytes(envp + 4, rp);
   QMLR_REQUIRE(smem <= 227 * 1024, "max_env too large for shared memory");
   cudaStream_t st = as_stream(stream);
-  const size_t wide = periodic_vjp_wide_smem(envp, rp);
-  if (wide_periodic(max_env) && wide <= kPeriodicWideMax) {
+  const long from = periodic_wide_from(9.0, 900.0, n_atoms);
+  const bool wide = may_be_wide(from, max_env, n_atoms);
+  if (wide) {   // (less shared memory than required above)
     QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_periodic_vjp_wide_kernel, kPeriodicWideMax));
-    fchl19_periodic_vjp_wide_kernel<<<n_atoms, 32 * kWideWarps, wide, st>>>(
-        coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, grad_rep, rep_ld, contrib,
+    fchl19_periodic_vjp_wide_kernel<<<n_atoms, 32 * kWideWarps, periodic_vjp_wide_smem(envp, rp), st>>>(
+        coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, grad_rep, rep_ld, contrib, from,
         device_error_ptr());
-  } else {
+    QMLR_LAUNCH_CHECK();
+  }
+  if (!wide || from > 0) {
     QMLR_CUDA_TRY(smem_attr_once((const void*)fchl19_periodic_vjp_kernel, 227 * 1024));
     fchl19_periodic_vjp_kernel<<<(n_atoms + kWarpsVjp - 1) / kWarpsVjp, 32 * kWarpsVjp, smem, st>>>(
         coords, elem, n_atoms, cell, env_ptr, env_atom, env_shift, max_env, envp, c, grad_rep, rep_ld, contrib,
-        device_error_ptr());
+        wide ? from : kNeverWide, device_error_ptr());
+    QMLR_LAUNCH_CHECK();
   }
-  QMLR_LAUNCH_CHECK();
   periodic_reduce_kernel<<<(3 * n_atoms + 255) / 256, 256, 0, st>>>(n_atoms, env_ptr, rev_ptr, rev_entry, contrib,
                                                                     scale, accumulate, grad_coords);
   QMLR_LAUNCH_CHECK();
