@@ -406,7 +406,8 @@ int qmlr_sorf_grad(const float* x, int32_t d, const int32_t* mol_ptr, int32_t n_
  * accumulation): x is split per atom into two FP16 parts after a power-of-two
  * row scale (2^-22 relative per element), the backward operand
  * alpha * sin(u) likewise with one power-of-two scale for all features; the
- * backward accumulator is promoted into FP32 sums every 4 stacks.
+ * backward accumulator is promoted into FP32 sums every 4 stacks (every 2, or
+ * every stack, where the number of stacks is not a multiple of 4, or of 2).
  * Phases use the same reduction and range check as qmlr_sorf (device error 6).
  *
  *   qmlr_sorf_tc_table_bytes(N_F)   bytes of the chain tables (4 N_F d bytes)
@@ -437,7 +438,8 @@ int qmlr_sorf_grad_tc(const float* x, int32_t d, const int32_t* mol_ptr, int32_t
 /*
  * Energy rows Z_m = sqrt(2/N_F) sum_{I in m} cos(u(x_I)) (SORF section; the
  * rows of the normal equations) with the forward chains on the tensor cores:
- * the same FP16 tables, operand split, phases and range check as
+ * the same FP16 tables, operand split (the low part carries the mean truncation
+ * of the accumulator and the rounding of c besides), phases and range check as
  * qmlr_sorf_grad_tc, cos of the phases, and each molecule's atoms added in
  * atom order in FP32 (the order of qmlr_sorf's PER_MOL mode), so Z_m does not
  * depend on the batch the molecule is in. A CTA of the persistent kernel takes
@@ -467,7 +469,7 @@ int qmlr_sorf_segment_sum_sin_tc(const float* x, int32_t d, const int32_t* mol_p
 /*
  * Force rows (as qmlr_force_rows: same rows, same order of the sum over the
  * centres) with the linear map of the projected Jacobian rows on the tensor
- * cores: the FP16 tables and operand split of qmlr_sorf_grad_tc.
+ * cores: the FP16 tables and operand split of qmlr_sorf_segment_sum_tc.
  *   n_jac_rows  rows of `tangents` (= jac_ptr[n_mol], 3 M^2 per molecule)
  *   sin_t       float [N_F/128][n_atoms][128] from qmlr_sorf_segment_sum_sin_tc
  *   work        qmlr_force_rows_tc_workspace_bytes(n_jac_rows) bytes, 256-byte

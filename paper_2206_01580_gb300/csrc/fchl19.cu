@@ -2086,8 +2086,9 @@ static bool may_be_wide(long wide_from, int max_env, int n_atoms) {
 }
 constexpr long kNeverWide = 1L << 62;
 
-// Batches whose atoms get a CTA each instead of a warp (forward and adjoint):
-// molecules of 64 atoms or more may occur and the mean says that they do. A
+// Batches whose atoms all get a CTA each instead of a warp (forward and adjoint; the
+// adjoint of other batches gives the centres of large molecules a CTA each all the
+// same): molecules of 64 atoms or more may occur and the mean says that they do. A
 // warp walks the ~10 000 pairs of a 200-atom molecule's centre alone, so mixed
 // sizes end in a tail: 5-200 atoms, 1606 in all, forward 495 -> 131 us and
 // adjoint 490 -> 130 us; 30 700 atoms 3.6 -> 2.3 ms and 4.0 -> 2.5 ms; 83 400
