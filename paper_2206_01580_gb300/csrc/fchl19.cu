@@ -763,7 +763,6 @@ fchl19_forward_reg_kernel(const float* __restrict__ coords, const int32_t* __res
 // VJP: one CTA per molecule, warps over centre atoms.
 
 struct VjpWarp {
-  float4* stage;  // [64] one chunk of pair contributions (atom index bits, gradient)
   float4* nb_u;   // [mxp]
   float4* nb_2b;  // [mxp]
   float* g;       // [rp]   gradient row of the centre
@@ -772,7 +771,7 @@ struct VjpWarp {
   int* nb_idx;    // [mxp]
 };
 __host__ __device__ __forceinline__ size_t vjp_warp_bytes(int mxp, int rp) {
-  return 64 * 16 + (size_t)mxp * (16 + 16 + 12 + 4 + 4) + (size_t)(rp + 4) * 4;
+  return (size_t)mxp * (16 + 16 + 12 + 4 + 4) + (size_t)(rp + 4) * 4;
 }
 
 // The centre's gradient row in the warp's buffer, the three-body columns moved
@@ -788,8 +787,7 @@ __device__ __forceinline__ const float2* grad3(const float* g, const Fchl19Const
 }
 __device__ __forceinline__ VjpWarp carve_vjp(char* base, int mxp, int rp) {
   VjpWarp s;
-  s.stage = reinterpret_cast<float4*>(base);
-  s.nb_u = s.stage + 64;
+  s.nb_u = reinterpret_cast<float4*>(base);
   s.nb_2b = s.nb_u + mxp;
   s.g = reinterpret_cast<float*>(s.nb_2b + mxp);
   s.facc = s.g + rp + 4;
@@ -1580,7 +1578,6 @@ __device__ __forceinline__ void vjp_wide_centre(const float* __restrict__ coords
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float4* pos = reinterpret_cast<float4*>(smem_raw);
   VjpWarp s;
-  s.stage = nullptr;
   s.nb_u = pos + mxp;
   s.nb_2b = s.nb_u + mxp;
   s.g = reinterpret_cast<float*>(s.nb_2b + mxp);
@@ -1989,7 +1986,6 @@ fchl19_periodic_vjp_wide_kernel(const float* __restrict__ coords, const int32_t*
   const long E = __ldg(env_ptr + n_atoms);
   if (E < wide_from) return;
   VjpWarp s;
-  s.stage = nullptr;
   s.nb_u = reinterpret_cast<float4*>(smem_raw);
   s.nb_2b = s.nb_u + envp;
   s.g = reinterpret_cast<float*>(s.nb_2b + envp);
